@@ -896,37 +896,37 @@ __device__ __noinline__ void hvp_sum(const MechView m, const Lane L, double invp
       }
       q = q0;
       tq = tq0;
-      double mkf = kf, mkr = kr, s1m = 0.0, wkm = 0.0;   // tb: sum_i s1_i dM_i / M, sum_i w_T dM_i / M
+      double mkf = kf, mkr = kr, s1m = 0.0, wkm = 0.0;   // tb: sum_i s1_i dM_i, sum_i w_T,i dM_i
       if (tb) {
-        const double invM = 1.0 / M.v;
+        // by the product rule: M may be zero (no species of the cell is a third body)
         allc.v = q0;
         q = M.v * q0;
         tq = M.v * tq0;
-        dG = fma(M.v, dG, q);
 #pragma unroll
         for (int i = 0; i < ND; ++i) {
-          allc.d[i] = qd[i];
-          const double ml = M.d[i] * invM;
-          qd[i] = fma(q, ml, M.v * qd[i]);
-          tqd[i] = fma(tq, ml, M.v * tqd[i]);
-          dGd[i] = fma(M.v, dGd[i], fma(dG - q, ml, qd[i]));
-          s1m = fma(s1[i], ml, s1m);
-          wkm = fma(wK[i], ml, wkm);
+          const double qd0 = qd[i];
+          allc.d[i] = qd0;
+          qd[i] = fma(q0, M.d[i], M.v * qd0);
+          tqd[i] = fma(tq0, M.d[i], M.v * tqd[i]);
+          dGd[i] = fma(M.v, dGd[i], fma(dG, M.d[i], qd[i]));
+          s1m = fma(s1[i], M.d[i], s1m);
+          wkm = fma(wK[i], M.d[i], wkm);
         }
+        dG = fma(M.v, dG, q);
         mkf *= M.v;
         mkr *= M.v;
       }
       double s1t = 0.0;
 #pragma unroll
       for (int i = 0; i < ND; ++i) s1t = fma(s1[i], tau[i], s1t);
-      // a slot's g = k O (O the other factors): sum_i s1_i g.d_i = k sum s1 O.d + g.v (theta s1t + s1m)
+      // a slot's g = M k O (O the other factors): sum_i s1_i g.d_i = M k sum s1 O.d + k O (M theta s1t + s1m)
 #pragma unroll
       for (int s = 0; s < 2 * kMaxSide; ++s) {
         const bool fw = s < kMaxSide;
         const int j = fw ? s : s - kMaxSide;
         if (fw ? j < x.nf() : (x.rev() && j < x.nb())) {
           const int k = fw ? x.fi(j) : x.bi(j), o = fw ? x.fo(j) : x.bo(j), n = fw ? x.nf() : x.nb();
-          const double kk = fw ? mkf : -mkr, theta = fw ? beta : gamma;
+          const double k1 = fw ? kf : -kr, kk = fw ? mkf : -mkr, theta = fw ? beta : gamma;
           double Ov, s1o, wko;
           const int other = 1 - j;   // of a two-species side
           if (n == 1 && o == 1) {
@@ -953,13 +953,14 @@ __device__ __noinline__ void hvp_sum(const MechView m, const Lane L, double invp
               wko = fma(wK[i], O.d[i], wko);
             }
           }
-          const double gv = (n == 1 && o == 1) ? kk : kk * Ov;
-          double a = fma(theta, s1t, s1m), b = fma(theta, wkt, wkm);
-          if (!tb) {
-            a = theta * s1t;
-            b = theta * wkt;
+          const double g1 = (n == 1 && o == 1) ? k1 : k1 * Ov, gv = tb ? M.v * g1 : g1;
+          double a = theta * s1t, b = theta * wkt;
+          if (tb) {
+            const double mt = M.v * theta;
+            a = fma(mt, s1t, s1m);
+            b = fma(mt, wkt, wkm);
           }
-          slot(k, gv, fma(kk, s1o, gv * a), fma(kk, wko, gv * b));
+          slot(k, gv, fma(kk, s1o, g1 * a), fma(kk, wko, g1 * b));
         }
       }
       phiq_v = q;

@@ -1,0 +1,151 @@
+// The device arithmetic of the thread-per-cell kernels compiled for the CPU, one lane at a
+// time, so that its numbers, and what they do on rare states, can be tested without a GPU:
+//   host_kernels <command> <mechanism file of 9 species> < doubles > doubles
+// The CUDA keywords are defined away; the few intrinsics the sources use are given here.
+#include <cmath>
+#include <cstdint>
+#include <cstdio>
+#include <cstring>
+#include <fstream>
+#include <iterator>
+#include <string>
+#include <vector>
+
+#define __CUDACC_RTC__
+#define __device__
+#define __host__
+#define __global__
+#define __forceinline__ inline
+#define __noinline__
+#define __launch_bounds__(...)
+#define __align__(n) __attribute__((aligned(n)))
+#define __shared__
+static inline long long __double_as_longlong(double x) {
+  long long b;
+  std::memcpy(&b, &x, 8);
+  return b;
+}
+static inline double __longlong_as_double(long long b) {
+  double x;
+  std::memcpy(&x, &b, 8);
+  return x;
+}
+static inline double rcbrt(double x) { return 1.0 / std::cbrt(x); }
+static inline double rsqrt(double x) { return 1.0 / std::sqrt(x); }
+static inline int min(int a, int b) { return a < b ? a : b; }
+static inline long long min(long long a, long long b) { return a < b ? a : b; }
+static inline int max(int a, int b) { return a > b ? a : b; }
+static inline long long max(long long a, long long b) { return a > b ? a : b; }
+using std::fma;
+using std::fmax;
+using std::fmin;
+using std::isfinite;
+using std::sqrt;
+struct int4 { int x, y, z, w; };
+// warp and block operations of the kernel bodies, which are not run here
+static struct { int x; } threadIdx, blockIdx, blockDim, gridDim;
+static inline void __syncthreads() {}
+static inline int __syncthreads_or(int v) { return v; }
+static inline int __any_sync(unsigned, bool v) { return v; }
+static inline unsigned __ballot_sync(unsigned, bool v) { return v; }
+template <class T>
+static inline T __shfl_sync(unsigned, T v, int) { return v; }
+static inline int __ffs(unsigned v) { return __builtin_ffs((int)v); }
+static inline int __popc(unsigned v) { return __builtin_popcount(v); }
+template <class T>
+static inline T atomicAdd(T* p, T v) { T o = *p; *p += v; return o; }
+template <class T>
+static inline T atomicMax(T* p, T v) { T o = *p; if (v > o) *p = v; return o; }
+static inline long long clock64() { return 0; }
+namespace rde {
+static inline bool recip_in_range(double x) {
+  const double a = std::fabs(x);
+  return a >= 0x1p-1022 && a < 0x1p1021;
+}
+static inline double recip(double x) { return 1.0 / x; }
+}  // namespace rde
+
+#include "chem_adjoint_body.cuh"
+#include "mech_host.h"
+
+using namespace rde;
+
+namespace {
+constexpr int K = 9, N = K + 1;
+
+FixThermo g_fix;
+
+// the packed reaction records with the fixed-point thermo of a specialised kernel
+struct FixReactions {
+  static constexpr unsigned kInert = 0u;
+  static constexpr bool kFix = true;
+  static int kCpBits, kDcpBits;
+  static bool two_ranges(int) { return true; }
+  static uint64_t th(int k, int r, int j) { return (uint64_t)g_fix.c[(size_t)(k * 2 + r) * 21 + j] + kFixBias; }
+  template <class F>
+  static void each(const MechView& m, F&& f) { GenericReactions::each(m, f); }
+};
+int FixReactions::kCpBits = 0;
+int FixReactions::kDcpBits = 0;
+
+std::vector<double> read_doubles() {
+  std::vector<double> v;
+  double x;
+  while (std::fread(&x, 8, 1, stdin) == 1) v.push_back(x);
+  return v;
+}
+void put(const double* p, size_t n) { std::fwrite(p, 8, n, stdout); }
+
+// in: invp, y[N], u[4][N], w[4][N]; out: g[N], thA[R], thE[R] of hvp_sum and of jtw's
+// dual-number evaluations summed over the stages
+template <class RX>
+void hvp(const MechView& m, const double* in) {
+  const int R = m.hdr->R;
+  std::vector<double> slots((size_t)(18 * K + 64) * kLaneThreads), g(N, 0.0), A(R, 0.0), E(R, 0.0);
+  const Lane L{slots.data()};
+  const double *y = in + 1, *U = in + 1 + N, *W = in + 1 + 5 * N;
+  hvp_sum<K, 4, RX>(m, L, in[0], y, U, W, 0, 1, g.data(), A.data(), E.data(), 1);
+  put(g.data(), N);
+  put(A.data(), R);
+  put(E.data(), R);
+  std::vector<double> s(N, 0.0), part(N, 0.0);
+  std::fill(A.begin(), A.end(), 0.0);
+  std::fill(E.begin(), E.end(), 0.0);
+  for (int st = 0; st < 4; ++st) {
+    Dual yd[N];
+    for (int i = 0; i < N; ++i) yd[i] = mk(y[i], U[st * N + i]);
+    jtw<K, GenericReactions>(m, L, 0, in[0], yd, W + st * N, part.data(), A.data(), E.data(), 1);
+    for (int i = 0; i < N; ++i) s[i] += part[i];
+  }
+  put(s.data(), N);
+  put(A.data(), R);
+  put(E.data(), R);
+}
+}  // namespace
+
+int main(int argc, char** argv) {
+  if (argc != 3) return 2;
+  std::ifstream f(argv[2], std::ios::binary);
+  const std::string text((std::istreambuf_iterator<char>(f)), std::istreambuf_iterator<char>());
+  std::vector<unsigned char> image;
+  std::string err;
+  if (pack_mechanism(text.data(), text.size(), &image, &err) != 0) {
+    std::fprintf(stderr, "%s\n", err.c_str());
+    return 3;
+  }
+  const MechView m = mech_view(image.data());
+  if (m.hdr->K != K) return 4;
+  const bool fixed = fix_thermo(m, &g_fix);
+  FixReactions::kCpBits = g_fix.cp_bits;
+  FixReactions::kDcpBits = g_fix.dcp_bits;
+  const std::vector<double> in = read_doubles();
+  const std::string cmd = argv[1];
+  if (cmd == "hvp" || cmd == "hvp_fix") {
+    if (in.size() != 1 + 9 * (size_t)N) return 5;
+    if (cmd == "hvp") hvp<GenericReactions>(m, in.data());
+    else if (fixed) hvp<FixReactions>(m, in.data());
+    else return 6;
+    return 0;
+  }
+  return 7;
+}

@@ -1,0 +1,68 @@
+"""The thread-per-cell kernels' device arithmetic on the CPU (tests/host/host_kernels.cpp):
+rare states and numerical properties that need no GPU."""
+import copy
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_2508_16105_gb300 import synth
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+CSRC = os.path.join(os.path.dirname(HERE), "paper_2508_16105_gb300", "csrc")
+
+
+@pytest.fixture(scope="session")
+def host(tmp_path_factory):
+    """run(command, mechanism, doubles) -> doubles"""
+    d = tmp_path_factory.mktemp("host")
+    exe = str(d / "host_kernels")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-w", "-ffp-contract=off", "-I", CSRC,
+                    os.path.join(HERE, "host", "host_kernels.cpp"), os.path.join(CSRC, "mech_host.cpp"), "-o", exe],
+                   check=True)
+
+    def run(command, mech, x):
+        path = str(d / "mech.txt")
+        with open(path, "w") as f:
+            f.write(mech.to_text())
+        r = subprocess.run([exe, command, path], input=np.ascontiguousarray(x, dtype=np.float64).tobytes(),
+                           stdout=subprocess.PIPE, check=True)
+        return np.frombuffer(r.stdout)
+
+    return run
+
+
+@pytest.fixture(scope="module")
+def no_collider():
+    """H2/air whose first three-body reaction takes no part from the species of air."""
+    mech = copy.deepcopy(synth.h2_air_mechanism(16105))
+    rx = next(r for r in mech.reactions if r.kind == "THREEBODY")
+    rx.eff = dict(rx.eff, N2=0.0, O2=0.0)
+    return mech
+
+
+@pytest.mark.parametrize("command", ["hvp", "hvp_fix"])
+@pytest.mark.parametrize("gas", ["N2", "air", "field"])
+def test_second_derivatives_without_a_third_body(host, no_collider, gas, command):
+    """hvp_sum equals the sum of its directions' dual-number evaluations, also where a third
+    body's concentration is exactly zero (pure N2 with a zero efficiency)."""
+    mech, N = no_collider, no_collider.K + 1
+    for seed in range(4):
+        if gas == "field":
+            c = synth.uniform_cells(mech, 1, seed=seed)
+            p, y = c.p[0], np.concatenate([c.Y[:, 0], c.T])
+        else:
+            p, y = 1e5 * (1 + seed), np.zeros(N)
+            y[mech.index("N2")] = 1.0 if gas == "N2" else 0.767
+            y[mech.index("O2")] = 1.0 - y[mech.index("N2")]
+            y[-1] = 700.0 + 400.0 * seed
+        u = synth.normal(seed, "u", 4 * N) * np.tile(np.append(np.full(N - 1, 1e-3), 10.0), 4)
+        w = synth.normal(seed, "w", 4 * N) * np.tile(np.append(np.ones(N - 1), 1e-3), 4)
+        out = host(command, mech, np.concatenate([[1.0 / p], y, u, w]))
+        assert np.isfinite(out).all()
+        # the same terms in another order: N + 2 R sums of some 10^3 rounded terms, whose
+        # cancellation leaves at least 10^-2 of the largest term: 10^3 2^-53 10^2 < 2e-11
+        a, b = out.reshape(2, -1)
+        for q in (slice(0, N), slice(N, N + mech.R), slice(N + mech.R, None)):
+            assert np.abs(a[q] - b[q]).max() <= 2e-11 * np.abs(b[q]).max()
