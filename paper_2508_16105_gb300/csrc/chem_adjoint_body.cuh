@@ -404,6 +404,7 @@ __device__ __forceinline__ RhsCtx adj_species(const MechView& m, Lane L, const d
     dcp_of(k, dcp, yw);
   }
   cx.lnPRT = kLnPstdOverRu - cx.lnT;
+  if (!cx.fix) cx.zs = max(cx.zs, fix_shift(cx.lnPRT));
   cx.zPRT = log2_fix(cx.lnPRT, cx.zs) + kParkBias;
   if (!cx.fix) {
 #pragma unroll

@@ -121,6 +121,20 @@ void hvp(const MechView& m, const double* in) {
   put(A.data(), R);
   put(E.data(), R);
 }
+
+// in: (invp, y[N]) per state; out: f[N] per state, once without and once with the Jacobian
+template <class RX>
+void rhs(const MechView& m, const std::vector<double>& in) {
+  std::vector<double> slots((size_t)Slots<K>::TOTAL * kLaneThreads);
+  const Lane L{slots.data()};
+  for (size_t at = 0; at < in.size(); at += 1 + N)
+    for (int jac = 0; jac < 2; ++jac) {
+      for (int i = 0; i < N; ++i) L[Slots<K>::ARG + i] = in[at + 1 + i];
+      if (jac) RhsOf<RX>::template eval<K, true, Slots<K>>(m, L, in[at]);
+      else RhsOf<RX>::template eval<K, false, Slots<K>>(m, L, in[at]);
+      for (int i = 0; i < N; ++i) put(&L[Slots<K>::VEC + i], 1);
+    }
+}
 }  // namespace
 
 int main(int argc, char** argv) {
@@ -144,6 +158,13 @@ int main(int argc, char** argv) {
     if (in.size() != 1 + 9 * (size_t)N) return 5;
     if (cmd == "hvp") hvp<GenericReactions>(m, in.data());
     else if (fixed) hvp<FixReactions>(m, in.data());
+    else return 6;
+    return 0;
+  }
+  if (cmd == "rhs" || cmd == "rhs_fix") {
+    if (in.size() % (1 + N)) return 5;
+    if (cmd == "rhs") rhs<GenericReactions>(m, in);
+    else if (fixed) rhs<FixReactions>(m, in);
     else return 6;
     return 0;
   }

@@ -13,12 +13,10 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(os.path.dirname(HERE), "paper_2508_16105_gb300", "csrc")
 
 
-@pytest.fixture(scope="session")
-def host(tmp_path_factory):
+def _build(d, *flags):
     """run(command, mechanism, doubles) -> doubles"""
-    d = tmp_path_factory.mktemp("host")
     exe = str(d / "host_kernels")
-    subprocess.run(["g++", "-std=c++17", "-O1", "-w", "-ffp-contract=off", "-I", CSRC,
+    subprocess.run(["g++", "-std=c++17", "-O1", "-w", "-ffp-contract=off", *flags, "-I", CSRC,
                     os.path.join(HERE, "host", "host_kernels.cpp"), os.path.join(CSRC, "mech_host.cpp"), "-o", exe],
                    check=True)
 
@@ -31,6 +29,18 @@ def host(tmp_path_factory):
         return np.frombuffer(r.stdout)
 
     return run
+
+
+@pytest.fixture(scope="session")
+def host(tmp_path_factory):
+    return _build(tmp_path_factory.mktemp("host"))
+
+
+@pytest.fixture(scope="session")
+def host_checked(tmp_path_factory):
+    """The same, ended by undefined integer arithmetic (shift counts, signed overflow)."""
+    return _build(tmp_path_factory.mktemp("checked"), "-fsanitize=shift,signed-integer-overflow",
+                  "-fsanitize-undefined-trap-on-error")
 
 
 @pytest.fixture(scope="module")
@@ -66,3 +76,18 @@ def test_second_derivatives_without_a_third_body(host, no_collider, gas, command
         a, b = out.reshape(2, -1)
         for q in (slice(0, N), slice(N, N + mech.R), slice(N + mech.R, None)):
             assert np.abs(a[q] - b[q]).max() <= 2e-11 * np.abs(b[q]).max()
+
+
+@pytest.mark.parametrize("command", ["rhs", "rhs_fix"])
+def test_integer_arithmetic_is_defined(host_checked, command):
+    """The fixed-point logarithms on ordinary states and on a Rosenbrock stage's wild ones:
+    |ln k| of 256 and more, temperatures of any finite size, thermo of next to nothing."""
+    mech = synth.h2_air_mechanism(16105)
+    flat = copy.deepcopy(mech)
+    for x in flat.species:
+        x.lo = x.hi = [0.5] + [0.0] * 6
+    for m in (mech, flat):
+        c = synth.uniform_cells(m, 32, seed=44)
+        states = [np.concatenate([[1.0 / c.p[i]], c.Y[:, i], [T]]) for i in range(32)
+                  for T in (c.T[i], 1e-280, 1e-3, 40.0, 130.0, 8191.0, 8193.0, 1e9, 1e120, 1e300)]
+        host_checked(command, m, np.concatenate(states))
