@@ -262,14 +262,15 @@ __device__ MixT<S> rhs_block(const MechView& m, const PlanView& pl, const CellT<
     // D = d omega / d c (fixed T): A_k plus the entry's terms in a fixed order
     for (int e = tid; e < K * K; e += kLT) {
       const PlanEntry en = pl.ent[e];
-      const int k = en.kj >> 16, last = pl.ent[e + 1].first;
+      const int k = (en.kj >> 6) & 63, last = pl.ent[e + 1].first;
+      const double* coef = pl.coef + (en.kj >> 12) * kPlanPage;
       S d = c.BK[k];
 #pragma unroll 4
       for (int q = en.first; q < last; ++q) {
         const uint32_t u = pl.con[q];
-        d += pl.coef[u >> 16] * c.RS[u & 0xffffu];
+        d += coef[u >> 16] * c.RS[u & 0xffffu];
       }
-      c.MX[k * c.LD + (en.kj & 0xffff)] = d;
+      c.MX[k * c.LD + (en.kj & 63)] = d;
     }
   }
   __syncthreads();

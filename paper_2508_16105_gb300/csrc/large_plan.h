@@ -6,10 +6,12 @@
 //   omega_k     = sum_{e in spr[k]} nu_e q_{r_e}                 (also d omega_k / dT)
 //   D[k][j]     = A_k + sum_{q in ent(k,j)} coef_q RS[r_q][slot_q]
 //   A_k         = sum_{e in row[k]} nu_e allc_{r_e}              (third-body / falloff [M] term, all j)
-// A term is one word: the index of its value in RS (low half) and of its coefficient in a
-// table of the distinct coefficients (high half).  The K * K entries of D come by falling
-// number of terms, so that the lanes of a warp loop equally long, each as one int2: k and j,
-// and the first term.  At 53 species and 325 reactions the lists take 50 KB, which the L1
+// A term is one word: the index of its value in RS (low half; the kernel's shared memory
+// bounds 9 R far below 65,536) and of its coefficient in a table of the distinct
+// coefficients (high half).  Where there are more than 65,536 of them (a thousand reactions
+// each with its own efficiencies), an entry of D counts its indices from its own page of the
+// table.  The K * K entries of D come by falling number of terms, so that the lanes of a warp
+// loop equally long, each as one int2: page, k and j, and the first term.  At 53 species and 325 reactions the lists take 50 KB, which the L1
 // beside three CTAs' shared memory holds (83 KB of terms in three arrays did not): 456 cells
 // 74.9 -> 70.8 ms, the adjoint's 152 cells 81.1 -> 71.8 ms.
 // where RS[r] holds the reaction's per-side derivatives (slots 0-2 forward, 3-5
@@ -37,8 +39,9 @@ struct PlanHeader {
 };
 static_assert(sizeof(PlanHeader) % 16 == 0, "plan header alignment");
 
+constexpr int kPlanPage = 4096;   // coefficients of a page
 struct PlanEntry {
-  int32_t kj;     // k << 16 | j
+  int32_t kj;     // page << 12 | k << 6 | j
   int32_t first;  // its first term; the next entry's `first` ends the list
 };
 

@@ -1,6 +1,7 @@
 // The device arithmetic of the thread-per-cell kernels compiled for the CPU, one lane at a
 // time, so that its numbers, and what they do on rare states, can be tested without a GPU:
-//   host_kernels <command> <mechanism file of 9 species> < doubles > doubles
+//   host_kernels <command> <mechanism file> < doubles > doubles
+// (9 species, except for the gather plan of the CTA-per-cell kernels).
 // The CUDA keywords are defined away; the few intrinsics the sources use are given here.
 #include <cmath>
 #include <cstdint>
@@ -66,6 +67,7 @@ static inline double recip(double x) { return 1.0 / x; }
 }  // namespace rde
 
 #include "chem_adjoint_body.cuh"
+#include "large_plan.h"
 #include "mech_host.h"
 
 using namespace rde;
@@ -135,6 +137,28 @@ void rhs(const MechView& m, const std::vector<double>& in) {
       for (int i = 0; i < N; ++i) put(&L[Slots<K>::VEC + i], 1);
     }
 }
+
+// the terms of the CTA-per-cell kernels' gather plan as the device reads them:
+// (matrix row and column, or -1 - list and species; index into RS; coefficient)
+void plan_terms(const unsigned char* image) {
+  std::vector<unsigned char> plan;
+  build_large_plan(image, &plan);
+  const PlanView pl = plan_view(plan.data());
+  const int KP = mech_view(image).hdr->K;
+  auto term = [&](double row, double col, uint32_t u, const double* coef) {
+    const double t[4] = {row, col, (double)(u & 0xffffu), coef[u >> 16]};
+    put(t, 4);
+  };
+  for (int k = 0; k < KP; ++k) {
+    for (int e = pl.spr_ptr[k]; e < pl.spr_ptr[k + 1]; ++e) term(-1, k, pl.spr[e], pl.coef);
+    for (int e = pl.row_ptr[k]; e < pl.row_ptr[k + 1]; ++e) term(-2, k, pl.row[e], pl.coef);
+  }
+  for (int e = 0; e < KP * KP; ++e) {
+    const PlanEntry en = pl.ent[e];
+    for (int q = en.first; q < pl.ent[e + 1].first; ++q)
+      term((en.kj >> 6) & 63, en.kj & 63, pl.con[q], pl.coef + (en.kj >> 12) * kPlanPage);
+  }
+}
 }  // namespace
 
 int main(int argc, char** argv) {
@@ -148,12 +172,16 @@ int main(int argc, char** argv) {
     return 3;
   }
   const MechView m = mech_view(image.data());
+  const std::string cmd = argv[1];
+  if (cmd == "plan") {
+    plan_terms(image.data());
+    return 0;
+  }
   if (m.hdr->K != K) return 4;
   const bool fixed = fix_thermo(m, &g_fix);
   FixReactions::kCpBits = g_fix.cp_bits;
   FixReactions::kDcpBits = g_fix.dcp_bits;
   const std::vector<double> in = read_doubles();
-  const std::string cmd = argv[1];
   if (cmd == "hvp" || cmd == "hvp_fix") {
     if (in.size() != 1 + 9 * (size_t)N) return 5;
     if (cmd == "hvp") hvp<GenericReactions>(m, in.data());

@@ -91,3 +91,50 @@ def test_integer_arithmetic_is_defined(host_checked, command):
         states = [np.concatenate([[1.0 / c.p[i]], c.Y[:, i], [T]]) for i in range(32)
                   for T in (c.T[i], 1e-280, 1e-3, 40.0, 130.0, 8191.0, 8193.0, 1e9, 1e120, 1e300)]
         host_checked(command, m, np.concatenate(states))
+
+
+def many_efficiencies(n):
+    """n copies of a three-body reaction of the 53-species mechanism with seeded efficiencies."""
+    mech = copy.deepcopy(synth.large_mechanism(16105))
+    rx = next(r for r in mech.reactions if r.kind == "THREEBODY")
+    mech.reactions = []
+    for i in range(n):
+        x = copy.deepcopy(rx)
+        x.A = rx.A / n
+        a = synth.uniform_range(i, "efficiencies", mech.K, 0.0, 2.0)
+        x.eff = {s.name: float(a[k]) for k, s in enumerate(mech.species)}
+        mech.reactions.append(x)
+    return mech
+
+
+def expected_plan(mech):
+    """(row, column, value index, coefficient) of every term, as test_gather_plan reads them."""
+    out = []
+    for r, x in enumerate(mech.reactions):
+        net = {}
+        for sign, side in ((-1.0, x.reac), (1.0, x.prod)):
+            for s, n in side:
+                net[s] = net.get(s, 0.0) + sign * n
+        for s, nu in net.items():
+            if nu == 0.0:
+                continue
+            k = mech.index(s)
+            out.append((-1, k, 9 * r + 7, nu))
+            for first, side in ((0, x.reac), (3, x.prod)):
+                out += [(k, mech.index(t), 9 * r + first + q, nu) for q, (t, _) in enumerate(side)]
+            if x.kind != "ELEM":
+                out.append((-2, k, 9 * r + 6, nu))
+                out += [(k, mech.index(t), 9 * r + 6, nu * (a - 1.0)) for t, a in x.eff.items() if a != 1.0]
+    return np.array(sorted(out))
+
+
+@pytest.mark.parametrize("n", [0, 1300])
+def test_gather_plan(host, n):
+    """Every term of the CTA-per-cell kernels' sums, also where the mechanism has more
+    distinct coefficients than a term's 16 bits count (n three-body reactions, each with its
+    own efficiency of every species)."""
+    mech = many_efficiencies(n) if n else synth.large_mechanism(16105)
+    got = host("plan", mech, np.zeros(0)).reshape(-1, 4)
+    want = expected_plan(mech)
+    assert n == 0 or len(np.unique(want[:, 3])) > 65536
+    assert np.array_equal(np.array(sorted(map(tuple, got))), want)
