@@ -17,7 +17,7 @@
 extern "C" {
 #endif
 
-/* y[i] = f(x[i]) for i < n, f = exp (fn == 0) or natural log (fn == 1).
+/* y[i] = f(x[i]) for i < n, f = exp (fn == 0), natural log (fn == 1) or 1/x (fn == 2).
  *   on_device == 0: x, y are host arrays, evaluated on the host (synchronous);
  *   on_device == 1: x, y are device arrays, evaluated by a kernel on `stream`
  *                   (a cudaStream_t as void*); the call synchronises the stream.

@@ -614,7 +614,7 @@ int rde_selftest_batched_lu(int dmma, int64_t batch, int n, double* A, int32_t* 
 }
 
 int rde_selftest_math(int fn, int64_t n, const double* x, double* y, int on_device, void* stream) {
-  if (fn != 0 && fn != 1) return fail(RDE_ERR_ARG, "fn must be 0 (exp) or 1 (log)");
+  if (fn < 0 || fn > 2) return fail(RDE_ERR_ARG, "fn must be 0 (exp), 1 (log) or 2 (reciprocal)");
   if (on_device != 0 && on_device != 1) return fail(RDE_ERR_ARG, "on_device must be 0 or 1");
   if (n < 0) return fail(RDE_ERR_ARG, "n < 0");
   if (n == 0) return RDE_OK;
@@ -622,7 +622,8 @@ int rde_selftest_math(int fn, int64_t n, const double* x, double* y, int on_devi
   const unsigned long long* et = rde::exp2_table_host();
   const double* lt = rde::log_table_host();
   if (!on_device) {
-    for (int64_t i = 0; i < n; ++i) y[i] = fn == 0 ? rde::exp_tab(x[i], et) : rde::log_tab(x[i], lt);
+    for (int64_t i = 0; i < n; ++i)
+      y[i] = fn == 0 ? rde::exp_tab(x[i], et) : (fn == 1 ? rde::log_tab(x[i], lt) : rde::recip(x[i]));
     return RDE_OK;
   }
   cudaStream_t s = static_cast<cudaStream_t>(stream);

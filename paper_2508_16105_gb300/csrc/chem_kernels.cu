@@ -212,13 +212,15 @@ cudaError_t launch_order(const LaunchArgs& args, unsigned* counts, long long* or
 }
 }  // namespace rde
 
-// ---- test hook: the library's exp / log on device arrays ----
+// ---- test hook: the library's exp / log / reciprocal on device arrays ----
 namespace rde {
 namespace {
 __global__ void selftest_math_kernel(int fn, long long n, const double* x, double* y, const double* tabs) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  y[i] = fn == 0 ? exp_tab(x[i], reinterpret_cast<const unsigned long long*>(tabs)) : log_tab(x[i], tabs + kExpTabSize);
+  y[i] = fn == 0   ? exp_tab(x[i], reinterpret_cast<const unsigned long long*>(tabs))
+         : fn == 1 ? log_tab(x[i], tabs + kExpTabSize)
+                   : recip(x[i]);
 }
 }  // namespace
 

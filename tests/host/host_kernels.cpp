@@ -58,13 +58,6 @@ static inline T atomicAdd(T* p, T v) { T o = *p; *p += v; return o; }
 template <class T>
 static inline T atomicMax(T* p, T v) { T o = *p; if (v > o) *p = v; return o; }
 static inline long long clock64() { return 0; }
-namespace rde {
-static inline bool recip_in_range(double x) {
-  const double a = std::fabs(x);
-  return a >= 0x1p-1022 && a < 0x1p1021;
-}
-static inline double recip(double x) { return 1.0 / x; }
-}  // namespace rde
 
 #include "chem_adjoint_body.cuh"
 #include "large_plan.h"
