@@ -284,6 +284,9 @@ std::string jit_common(const unsigned char* image, const char* include, int grou
       }
       o << "},\n";
     }
+    o << "};\n"
+      << "static __device__ constexpr int kDcpBits[" << K << "] = {";
+    for (int k = 0; k < K; ++k) o << fix.dcp_bits[k] << ", ";
     o << "};\n";
   }
   unsigned long long two = 0;   // species whose two temperature ranges differ
@@ -296,7 +299,9 @@ std::string jit_common(const unsigned char* image, const char* include, int grou
   o << "struct Reactions {\n"
     << "  static constexpr unsigned kInert = " << inert << "u;\n"
     << "  static constexpr bool kFix = " << (fixed ? "true" : "false") << ";\n"
-    << "  static constexpr int kCpBits = " << fix.cp_bits << ", kDcpBits = " << fix.dcp_bits << ";\n"
+    << "  static constexpr int kCpBits = " << fix.cp_bits << ";\n"
+    << "  static __device__ __forceinline__ constexpr int dcp_bits(int k) { return " << (fixed ? "kDcpBits[k]" : "0")
+    << "; }\n"
     << "  static __device__ __forceinline__ constexpr bool two_ranges(int k) { return (" << two << "ull >> k) & 1ull; }\n"
     << "  static __device__ __forceinline__ uint64_t th(int k, int r, int j) { return "
     << (fixed ? "r ? kTh[k][1][j] : kTh[k][0][j]" : "0") << "; }\n"

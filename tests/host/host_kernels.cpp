@@ -74,14 +74,14 @@ FixThermo g_fix;
 struct FixReactions {
   static constexpr unsigned kInert = 0u;
   static constexpr bool kFix = true;
-  static int kCpBits, kDcpBits;
+  static int kCpBits;
+  static int dcp_bits(int k) { return g_fix.dcp_bits[k]; }
   static bool two_ranges(int) { return true; }
   static uint64_t th(int k, int r, int j) { return (uint64_t)g_fix.c[(size_t)(k * 2 + r) * 21 + j] + kFixBias; }
   template <class F>
   static void each(const MechView& m, F&& f) { GenericReactions::each(m, f); }
 };
 int FixReactions::kCpBits = 0;
-int FixReactions::kDcpBits = 0;
 
 std::vector<double> read_doubles() {
   std::vector<double> v;
@@ -131,6 +131,29 @@ void rhs(const MechView& m, const std::vector<double>& in) {
     }
 }
 
+// in: T per state; out, per state and species: Cp/R, the polynomial part of H/RT,
+// d(Cp/R)/dT and G/RT in fixed point, then the same in FP64
+void thermo(const MechView& m, const std::vector<double>& in) {
+  for (double T : in) {
+    RhsCtx cx{};
+    cx.invT = recip(T);
+    cx.lnT = log_tab(T, m.logtab);
+    cx.zlnT = (uint64_t)to_fix(cx.lnT, 59);
+    cx.zinvT = (uint64_t)to_fix(cx.invT, 70);
+    for (int k = 0; k < K; ++k) {
+      SpecPacked sp = m.sp[k];
+      sp.h[0][5] = sp.h[1][5] = 0.0;
+      double o[8], g;
+      int64_t z;
+      thermo_fix<true, FixReactions>(sp, k, T, (uint64_t)to_fix(T, 50), cx, o[0], o[1], z, o[2]);
+      o[3] = fix_to_log(z, 0);
+      thermo_fp64<true>(sp, T, cx.lnT, cx.invT, o[4], o[5], g, o[6]);
+      o[7] = g;
+      put(o, 8);
+    }
+  }
+}
+
 // the terms of the CTA-per-cell kernels' gather plan as the device reads them:
 // (matrix row and column, or -1 - list and species; index into RS; coefficient)
 void plan_terms(const unsigned char* image) {
@@ -173,7 +196,6 @@ int main(int argc, char** argv) {
   if (m.hdr->K != K) return 4;
   const bool fixed = fix_thermo(m, &g_fix);
   FixReactions::kCpBits = g_fix.cp_bits;
-  FixReactions::kDcpBits = g_fix.dcp_bits;
   const std::vector<double> in = read_doubles();
   if (cmd == "hvp" || cmd == "hvp_fix") {
     if (in.size() != 1 + 9 * (size_t)N) return 5;
@@ -187,6 +209,11 @@ int main(int argc, char** argv) {
     if (cmd == "rhs") rhs<GenericReactions>(m, in);
     else if (fixed) rhs<FixReactions>(m, in);
     else return 6;
+    return 0;
+  }
+  if (cmd == "thermo") {
+    if (!fixed) return 6;
+    thermo(m, in);
     return 0;
   }
   return 7;

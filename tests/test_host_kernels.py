@@ -138,3 +138,42 @@ def test_gather_plan(host, n):
     want = expected_plan(mech)
     assert n == 0 or len(np.unique(want[:, 3])) > 65536
     assert np.array_equal(np.array(sorted(map(tuple, got))), want)
+
+
+def fitted(low, high):
+    """The H2/air species with fits of the given two ranges, a0 as seeded."""
+    mech = copy.deepcopy(synth.h2_air_mechanism(16105))
+    for x in mech.species:
+        x.lo, x.hi = [x.lo[0]] + low + x.lo[5:], [x.hi[0]] + high + x.hi[5:]
+    return mech
+
+
+@pytest.mark.parametrize("fit", ["seeded", "wide", "narrow"])
+def test_fixed_point_thermo_is_no_coarser_than_fp64(host, fit):
+    """Cp/R, H/RT and d(Cp/R)/dT in fixed point against 80-bit arithmetic.  Coefficients of
+    the size of published fits (wide: those for 1,000 to 3,500 K, narrow: 200 to 1,000 K) have
+    too coarse a unit and stay in FP64."""
+    wide, narrow = [2.2e-3, -1.6e-7, -1.0e-10, 1.7e-14], [-2.0e-3, 6.5e-6, -5.5e-9, 1.8e-12]
+    mech = synth.h2_air_mechanism(16105) if fit == "seeded" else fitted(wide if fit == "wide" else narrow, wide)
+    T = synth.uniform_range(54, "T", 4000, 300.0, 3500.0)
+    try:
+        out = host("thermo", mech, T).reshape(len(T), mech.K, 8).astype(np.longdouble)
+    except subprocess.CalledProcessError as e:
+        assert e.returncode == 6 and fit != "seeded"      # refused: the kernels use FP64
+        return
+    x = T.astype(np.longdouble)
+    for k, s in enumerate(mech.species):
+        # the coefficients as the packed mechanism holds them (doubles)
+        rows = [np.array([[a[0], a[1], a[2], a[3], a[4]], [a[0], a[1] / 2, a[2] / 3, a[3] / 4, a[4] / 5],
+                          [a[1], 2 * a[2], 3 * a[3], 4 * a[4], 0.0]]).astype(np.longdouble) for a in (s.lo, s.hi)]
+        for q, name in enumerate(("Cp/R", "H/RT", "d(Cp/R)/dT")):
+            c = np.where((T >= s.Tmid)[:, None], rows[1][q], rows[0][q])
+            want = (((c[:, 4] * x + c[:, 3]) * x + c[:, 2]) * x + c[:, 1]) * x + c[:, 0]
+            ulp = np.spacing(np.abs(want).astype(np.float64)).astype(np.longdouble)
+            err = float((np.abs(out[:, k, q] - want) / ulp).max())
+            if name == "d(Cp/R)/dT":
+                # a unit is at most 2^-61 of the scheme's bound; three steps lose up to 6.1 units
+                bound = max(abs(a[j]) * j * 2.0 ** (14 * (j - 1)) for a in (s.lo, s.hi) for j in (1, 2, 3, 4)) * 2
+                assert err <= 0.5 + 6.1 * 2.0 ** -61 * bound / float(ulp.min()), (s.name, name, err)
+            else:
+                assert err <= 0.71, (s.name, name, err)   # 0.5 + 6.6 units of 2^-56 at Cp/R of 2 to 4
