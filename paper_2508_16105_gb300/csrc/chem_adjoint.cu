@@ -137,8 +137,8 @@ cudaError_t adjoint_k(const AdjArgs& a, cudaStream_t stream) {
   const bool self = a.ckpt_S > 0;
   const void* rev = self ? reinterpret_cast<const void*>(reverse_kernel<K, true>)
                          : reinterpret_cast<const void*>(reverse_kernel<K, false>);
-  cudaError_t e = cudaFuncSetAttribute(record_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_rec);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(rev, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_rev);
+  cudaError_t e = raise_shared_limit(reinterpret_cast<const void*>(record_kernel<K>), smem_rec);
+  if (e == cudaSuccess) e = raise_shared_limit(rev, smem_rev);
   if (e != cudaSuccess) return e;
   int fit_rec = 0, fit_rev = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit_rec, record_kernel<K>, kThreadsA, smem_rec);

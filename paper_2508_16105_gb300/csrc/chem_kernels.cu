@@ -4,6 +4,8 @@
 // ROS2); the body is in chem_kernel_body.cuh.
 #include <cuda_runtime.h>
 
+#include <mutex>
+
 #include "chem_kernel_body.cuh"
 
 namespace rde {
@@ -22,8 +24,7 @@ size_t smem_bytes(int mech_bytes, int n_blocks) {
 
 template <int K, bool QUEUE, int METHOD>
 cudaError_t set_smem(size_t smax) {
-  return cudaFuncSetAttribute(chem_advance_kernel<K, QUEUE, METHOD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)smax);
+  return raise_shared_limit(reinterpret_cast<const void*>(chem_advance_kernel<K, QUEUE, METHOD>), smax);
 }
 
 template <int K>
@@ -81,6 +82,15 @@ size_t kernel_shared_bytes(int K, int mech_bytes) {
     case 9: return smem_bytes<9>(mech_bytes, 0);
     default: return 0;
   }
+}
+
+cudaError_t raise_shared_limit(const void* kernel, size_t bytes) {
+  static std::mutex mu;   // the limit is read and written as one step
+  std::lock_guard<std::mutex> lk(mu);
+  cudaFuncAttributes at;
+  const cudaError_t e = cudaFuncGetAttributes(&at, kernel);
+  if (e != cudaSuccess || bytes <= (size_t)at.maxDynamicSharedSizeBytes) return e;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
 cudaError_t prepare_advance(int K, int mech_bytes, int* fit) {

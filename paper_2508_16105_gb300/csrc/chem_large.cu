@@ -225,7 +225,7 @@ cudaError_t prepare_large(int K, int R, int* fit) {
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (e != cudaSuccess) return e;
   if (smax > (size_t)optin) return cudaErrorInvalidConfiguration;
-  e = cudaFuncSetAttribute(chem_large_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smax);
+  e = raise_shared_limit(reinterpret_cast<const void*>(chem_large_kernel), smax);
   if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(fit, chem_large_kernel, kLT, smax);
   if (e == cudaSuccess && *fit < 1) e = cudaErrorInvalidConfiguration;
   return e;

@@ -570,9 +570,8 @@ cudaError_t prepare_large_adjoint(int K, int R) {
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (e != cudaSuccess) return e;
   if (smem > (size_t)optin) return cudaErrorInvalidConfiguration;
-  e = cudaFuncSetAttribute(chem_large_adjoint_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(chem_large_adjoint_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  e = raise_shared_limit(reinterpret_cast<const void*>(chem_large_adjoint_kernel<false>), smem);
+  if (e == cudaSuccess) e = raise_shared_limit(reinterpret_cast<const void*>(chem_large_adjoint_kernel<true>), smem);
   return e;
 }
 

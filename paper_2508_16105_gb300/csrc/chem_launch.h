@@ -41,6 +41,11 @@ struct LaunchArgs {
 // true if a kernel is compiled for K species
 bool kernel_supports(int K);
 
+// Raises a kernel's dynamic shared-memory limit on the current device to `bytes`.  The limit
+// belongs to the kernel, which serves every handle, so it is never lowered: a mechanism
+// loaded after a larger one leaves the room the larger one's launches need.
+cudaError_t raise_shared_limit(const void* kernel, size_t bytes);
+
 // Once per mechanism, outside any stream capture: raise the kernels' dynamic
 // shared-memory limit for this mechanism and report how many queue CTAs fit per SM.
 cudaError_t prepare_advance(int K, int mech_bytes, int* fit);
