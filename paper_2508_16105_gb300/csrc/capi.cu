@@ -452,32 +452,37 @@ cudaError_t launch_cells(const rde_mech_s* h, rde::LaunchArgs& a, bool large, cu
   a.park_lanes = h->park_lanes;
   return h->jit_ok ? rde::jit_launch(h->jit, a, s) : rde::launch_advance(a, s);
 }
-}  // namespace
-
-int rde_chem_advance_ex(rde_mech_t h, const rde_chem_call* c, void* stream) {
+// The checks of a step's arguments; reports the kernel (CTA per cell or not) and the cells.
+int check_call(rde_mech_s* h, const rde_chem_call* c, bool* large, long long* n_total) {
   if (!h || !c) return fail(RDE_ERR_NULL, "handle and call are required");
   if (!(c->dt > 0) || !std::isfinite(c->dt)) return fail(RDE_ERR_ARG, "dt must be finite and > 0");
   if (c->schedule != RDE_SCHED_AUTO && c->schedule != RDE_SCHED_PLAIN && c->schedule != RDE_SCHED_QUEUE &&
       c->schedule != RDE_SCHED_BLOCK)
     return fail(RDE_ERR_ARG, "unknown schedule");
-  bool large = false;
-  if (int prc = pick_kernel(h, c->schedule, &large)) return prc;
-  if (c->threads_per_cta == 256 && c->schedule != RDE_SCHED_PLAIN && !large && h->opt.method == RDE_METHOD_RODAS3)
+  if (int prc = pick_kernel(h, c->schedule, large)) return prc;
+  if (c->threads_per_cta == 256 && c->schedule != RDE_SCHED_PLAIN && !*large && h->opt.method == RDE_METHOD_RODAS3)
     h->wide_asked = true;
-  if (int trc = check_threads(h, c, large)) return trc;
+  if (int trc = check_threads(h, c, *large)) return trc;
   if (c->ctas_per_sm < 0 || c->ctas_per_sm > 32) return fail(RDE_ERR_ARG, "ctas_per_sm out of range");
-  long long n_total;
   if (c->blocks) {
     if (c->n_blocks < 1 || c->n_blocks > 1024) return fail(RDE_ERR_ARG, "n_blocks must be 1..1024");
     if (c->n_total < 0) return fail(RDE_ERR_ARG, "n_total < 0");
     if (!aligned8(c->blocks)) return fail(RDE_ERR_ALIGN, "block table must be 8-byte aligned");
-    n_total = c->n_total;
+    *n_total = c->n_total;
   } else {
     int rc = check_block(c->cells, h->K);
     if (rc) return rc;
-    n_total = c->cells.n;
+    *n_total = c->cells.n;
   }
   if (c->order && !aligned8(c->order)) return fail(RDE_ERR_ALIGN, "order must be 8-byte aligned");
+  return RDE_OK;
+}
+}  // namespace
+
+int rde_chem_advance_ex(rde_mech_t h, const rde_chem_call* c, void* stream) {
+  bool large = false;
+  long long n_total = 0;
+  if (int rc = check_call(h, c, &large, &n_total)) return rc;
   DeviceGuard g(h->device);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const bool ordered = orders_cells(h, c, n_total, large) && reserve_order(h, n_total, s);
@@ -709,16 +714,14 @@ struct rde_graph_s {
 int rde_chem_graph_create(rde_mech_t h, const rde_chem_call* c, int n_steps, void** out) {
   if (!h || !c || !out) return fail(RDE_ERR_NULL, "handle, call and out are required");
   if (n_steps < 1 || n_steps > 100000) return fail(RDE_ERR_ARG, "n_steps must be 1..100000");
+  bool large = false;
+  long long n_total = 0;
+  if (int crc = check_call(h, c, &large, &n_total)) return crc;
   DeviceGuard g(h->device);
   cudaStream_t s = nullptr;
   cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
   if (e != cudaSuccess) return cuda_fail(e, "create capture stream");
-  {
-    // room for the steps' cost order, before the capture begins
-    const long long n = c->blocks ? c->n_total : c->cells.n;
-    bool large = false;
-    if (pick_kernel(h, c->schedule, &large) == RDE_OK && orders_cells(h, c, n, large)) reserve_order(h, n, s);
-  }
+  if (orders_cells(h, c, n_total, large)) reserve_order(h, n_total, s);   // before the capture begins
   cudaGraph_t graph = nullptr;
   int rc = RDE_OK;
   e = cudaStreamBeginCapture(s, cudaStreamCaptureModeRelaxed);
