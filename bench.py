@@ -484,8 +484,8 @@ def adjoint_leg(mech, n: int) -> dict:
     T, Y = T0.clone(), Y0.clone()
 
     def fwd(threads=128):
-        # 128 threads: the arithmetic the adjoint's re-integration retraces (its n_acc sizes
-        # the recorded mode); 256: the fastest forward, for the second ratio
+        # 128 threads: the kernel the first ratio has always been taken against; 256: the
+        # default and fastest forward, for the second ratio (both give the same n_acc)
         T.copy_(T0)
         Y.copy_(Y0)
         rde_chem.rde_chem_advance_ex(m.handle, ADJ_DT, cells=rde_chem.make_block(p, T, Y, n_acc=n_acc),
@@ -493,7 +493,7 @@ def adjoint_leg(mech, n: int) -> dict:
 
     wide_ok = True
     try:
-        fwd(256)    # builds the wide kernel (untimed); its counts are replaced by the 128-thread pass
+        fwd(256)    # warm-up
     except rde_chem.RdeError:
         wide_ok = False
     fwd()
@@ -551,8 +551,8 @@ def adjoint_leg(mech, n: int) -> dict:
            "workspace_GB": (big if stages else small) / 1e9, "workspace_recompute_GB": small / 1e9,
            "adjoint_cell_steps_per_s": n / t_b,
            "forward_wide_s": t_w, "ratio_vs_wide_forward": (t_b / t_w) if t_w else None,
-           "forward_note": "forward_s: the 128-thread kernel, whose arithmetic the adjoint retraces; "
-                           "forward_wide_s: the wide 256-thread queue kernel, the fastest forward",
+           "forward_note": "forward_s: the 128-thread kernel; forward_wide_s: the wide 256-thread queue kernel, "
+                           "the default",
            "grad_norms": {"gT0": float(gT0.norm()), "glnA": float(glnA.norm()), "gE": float(gE.norm())}}
     m.close()
     del ws
@@ -753,9 +753,9 @@ def main():
             "traffic": traffic * n if traffic is not None else None,
             "peak_source": "FP64 2 DFMA/clk/SM x 152 SMs x 2070 MHz (recipe unit counts); DFMA microbenchmark "
                            "measured %.0f GFLOP/s" % roofline.FP64_MEASURED_GFLOPS,
-            "frac_note": "the count is the algorithm's FP64 work; exp, log, reciprocals and the thermodynamic "
-                         "polynomials run as exact 64-bit fixed point on the integer and FP32 pipes, so frac "
-                         "can pass 1 without the FP64 pipe being full",
+            "frac_note": "the algorithm's work over the FP64 peak, which is not the FP64 pipe's occupancy: exp, rate "
+                         "exponents, reciprocals and the thermodynamic polynomials run in 64-bit fixed point on the "
+                         "integer and FP32 pipes, so it can pass 1 without the FP64 pipe being full",
             "kernel": kname, "kernel_ms": 1e3 * k_avg,
             "flops_per_attempt": fl["total"], "flop_rule": "exp, log, division and root = 1 flop; FMA = 2",
             "attempts_per_launch": attempts,

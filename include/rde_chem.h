@@ -187,9 +187,10 @@ typedef struct {
  * warp per SM sub-partition (with one cell per resident CTA) orders them itself
  * by predicted cost (dt / h_hint where a hint is given, else T^2 p), longest
  * first: two short kernels before the step and 8 bytes per cell of device
- * memory that the handle keeps (grown on demand outside captures; inside one,
- * and in rde_chem_advance_noalloc, the queue runs in cell order unless the room
- * is there already).  A cell's result does not depend on the order.
+ * memory that the handle keeps (allocated when a call outgrows it, outside
+ * captures; inside one the queue runs in cell order unless the room is there
+ * already).  rde_chem_advance_noalloc runs in the caller's order or in cell order.
+ * A cell's result does not depend on the order.
  * The kernels read a device block table without the host checking it: a block
  * whose n is negative is treated as empty, and positions beyond the table's
  * total are never handed out. */
@@ -304,7 +305,8 @@ int rde_chem_advance_noalloc(rde_mech_t h, const rde_chem_call* c, void* stream)
  * if given, carried from step to step), for time loops such as the paper's 500 us
  * of simulated time split into flow steps (Section 3.2.2).  The call is captured
  * on an internal stream; the graph holds, per step, a memset of the handle's
- * scratch and one kernel launch, so replaying it costs one host call.
+ * scratch and one kernel launch (three where the library orders the queue), so
+ * replaying it costs one host call.
  *   c        the call to repeat (device arrays, block table, schedule, as in
  *            rde_chem_advance_ex); captured by value: the arrays it points to must
  *            stay valid while the graph exists
@@ -317,10 +319,11 @@ int rde_chem_graph_launch(void* graph, void* stream);
 /* Destroy the graph (NULL is a no-op). */
 int rde_chem_graph_destroy(void* graph);
 
-/* Launch shape of the 128-thread kernel that serves the handle's AUTO schedule
- * (thread per cell; CTA per cell where that is the only one): threads per CTA, queue CTAs that fit per SM, and dynamic
- * shared memory per CTA (bytes, without a block table).  Any argument may be
- * NULL. */
+/* Launch shape of the handle's 128-thread kernel (thread per cell; CTA per cell where
+ * that is the only one): threads per CTA, queue CTAs that fit per SM, and dynamic
+ * shared memory per CTA (bytes, without a block table).  It is the kernel of calls
+ * with threads_per_cta = 128; with 0 a queue call runs the wide kernel where the
+ * handle has it.  Any argument may be NULL. */
 int rde_chem_kernel_info(rde_mech_t h, int* threads_per_cta, int* max_ctas_per_sm, size_t* shared_bytes);
 
 /* ---- discrete adjoint ------------------------------------------------------
@@ -336,7 +339,7 @@ int rde_chem_kernel_info(rde_mech_t h, int* threads_per_cta, int* max_ctas_per_s
  * steps, and sweeps them backwards.  Kernels: thread per cell where a
  * thread-per-cell kernel serves the mechanism (precompiled for 2, 3 and 9
  * species, or specialised at load time), else, or with schedule =
- * RDE_SCHED_BLOCK, one CTA of 128 threads per cell for any K + 1 <= 64 (the
+ * RDE_SCHED_BLOCK, one CTA of 256 threads per cell for any K + 1 <= 64 (the
  * 53-species stress mechanism), which always recomputes the stages.
  *
  * rde_chem_advance_adjoint (below) is self-contained: it needs only the step's
@@ -371,9 +374,13 @@ int rde_chem_kernel_info(rde_mech_t h, int* threads_per_cta, int* max_ctas_per_s
  * only (recomputed stages are not bitwise those of the re-integration).  The
  * CTA-per-cell adjoint re-integrates with the CTA-per-cell step, so its n_steps
  * must come from a forward pass with RDE_SCHED_BLOCK (which is what AUTO takes for
- * such a mechanism).  The thread-per-cell adjoint re-integrates with the
- * operations of the thread-per-cell forward kernels, bit for bit, so n_steps may come
- * from any of them. */
+ * such a mechanism).  The specialised adjoint re-integrates with the operations of the
+ * specialised forward kernels (plain, 128-thread and wide), bit for bit, and the
+ * precompiled adjoint with those of the precompiled ones, so n_steps may come from any
+ * of the same kind.  Between the kinds only rounding differs (fixed point against FP64):
+ * with a specialised forward and a precompiled adjoint, which serves the handle if the
+ * adjoint's compilation fails, a cell whose step count changes gets
+ * RDE_CELL_ADJ_MISMATCH. */
 typedef struct {
   int64_t n;                 /* cells (single block) */
   const double* p;           /* [n] Pa */

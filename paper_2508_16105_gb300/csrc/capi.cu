@@ -49,8 +49,7 @@ struct rde_mech_s {
   size_t plan_offset = 0;   // gather plan behind the image in d_mech
   std::vector<unsigned char> image;  // host copy of the device tables
   std::vector<double> E_J;           // activation energies as given (J/mol)
-  // device scratch: [0] work-queue counter, [1..8) statistics
-  // queue counter, statistics (7 words) and the cost order's counters
+  // device scratch: work-queue counter, statistics (7 words) and the cost order's counters
   unsigned long long* d_scratch = nullptr;
   // the cost order of a call's cells: grown to twice its size or the call's on demand; the
   // buffers it outgrew stay until the handle goes, since graphs may hold them (together less

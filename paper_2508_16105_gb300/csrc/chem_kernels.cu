@@ -145,7 +145,8 @@ __device__ __forceinline__ int cost_bin(const LaunchArgs& a, const long long* of
     x = (float)(T * T * c.p[c.i]);
     base = 127 + 24;        // bins from 2^24 K^2 Pa to 2^56
   }
-  const int b = (int)(__float_as_uint(x) >> 21) - 4 * base;   // NaN and infinity: the last bin
+  const int b = (int)(__float_as_uint(x) >> 21) - 4 * base;
+  // infinity goes first, NaN and what is not positive last
   return x > 0.0f ? max(0, min(kOrderBins - 1, b)) : 0;
 }
 

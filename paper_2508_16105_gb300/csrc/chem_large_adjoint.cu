@@ -3,7 +3,7 @@
 // frozen sequence of accepted RODAS3 steps, as in chem_adjoint_body.cuh, for
 // mechanisms whose N x N matrix does not fit the thread-per-cell lane slots.
 //
-// One persistent CTA of 128 threads per cell (work queue; the cells come in the
+// One persistent CTA of 256 threads per cell (work queue; the cells come in the
 // cost order of order_kernel, most accepted steps first).  Per cell it
 //  1. re-integrates the cell with the forward kernel's attempt (large_attempt),
 //     writing the start state y_n and size h_n of every accepted step into the
@@ -238,7 +238,9 @@ __global__ void __launch_bounds__(kLT, 1) chem_large_adjoint_kernel(const AdjArg
   c.INVD = d; d += N;
   c.RS = d; d += 9 * R;
   c.red = d; d += 8;
-  long long* cellidx = reinterpret_cast<long long*>(c.red + 6);   // red[0..3] serve block_sum
+  // the sums of eight warps use all of red[0..7]; the cell index is handed out through
+  // red[6] between two barriers, after the barrier that ends the previous cell's last sum
+  long long* cellidx = reinterpret_cast<long long*>(c.red + 6);
   // the explicit Jacobian at a stage argument: the forward cell with its own matrix, in
   // the memory of the dual cell's matrix (the two are never live at the same time)
   Cell cj = c;
