@@ -177,3 +177,22 @@ def test_fixed_point_thermo_is_no_coarser_than_fp64(host, fit):
                 assert err <= 0.5 + 6.1 * 2.0 ** -61 * bound / float(ulp.min()), (s.name, name, err)
             else:
                 assert err <= 0.71, (s.name, name, err)   # 0.5 + 6.6 units of 2^-56 at Cp/R of 2 to 4
+
+
+def test_fixed_point_gibbs(host):
+    """G/RT as a fixed-point logarithm against 80-bit arithmetic.  Six Horner steps lose at most
+    3 units of 2^-51 each, halved by every later step in T (14 units in all, in base 2); ln T
+    is good to 2 ulp (2^-49), 1/T and the final product are rounded once."""
+    mech = synth.h2_air_mechanism(16105)
+    T = synth.uniform_range(55, "T", 4000, 150.0, 8000.0)
+    out = host("thermo", mech, T).reshape(len(T), mech.K, 8)
+    x = T.astype(np.longdouble)
+    for k, s in enumerate(mech.species):
+        g = [np.array([a[0] - a[6], -a[0], a[1] / 2 - a[1], a[2] / 3 - a[2] / 2, a[3] / 4 - a[3] / 3,
+                       a[4] / 5 - a[4] / 4, a[5]]).astype(np.longdouble) for a in (s.lo, s.hi)]
+        c = np.where((T >= s.Tmid)[:, None], g[1], g[0])
+        want = c[:, 0] + c[:, 1] * np.log(x) + x * (c[:, 2] + x * (c[:, 3] + x * (c[:, 4] + x * c[:, 5]))) + c[:, 6] / x
+        tol = (14 * 2.0 ** -51 * np.log(2.0) + np.abs(c[:, 1]) * 2.0 ** -49 + np.abs(c[:, 6] / x) * 2.0 ** -53 +
+               np.abs(want) * 2.0 ** -52)
+        err = np.abs(out[:, k, 3] - want)
+        assert (err <= tol).all(), (s.name, float((err / tol).max()))
